@@ -923,7 +923,7 @@ __device__ __forceinline__ int mig_consumer(MigSmem& S, const TT* data, const Ge
                 // two-way time, hundreds of samples, is in the FP64 reference).  One reciprocal root
                 // gives 1/R_a and R_a = q_a / R_a; the source leg's (dR_s, 1/R_s) is cached per source
                 // position.  The weight z (R_s + R_r) (1/R_s^2 + 1/R_r^2) / 2 (2D: sqrt(R_s R_r)) is 0 on
-                // the surface row, where zc's z / 2 is stored as 0 (every factor is finite)
+                // the surface row, where zc's z / 2 is stored as 0 (every factor is finite, see root_pair)
                 int aacls = 1;   // anti-aliasing classes as in the direct branch
                 if constexpr (AA) {
                     aacls = aa_class(g.aa_c, cxf - h.x, cyf - h.y, cxf - h.z, cyf - h.w, aa_lo, aa_hi, inside);
