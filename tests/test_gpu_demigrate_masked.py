@@ -1,4 +1,5 @@
-"""The adjoint where a lane or a point is to add nothing: times a hair past the last sample."""
+"""The adjoint where a lane or a point is to add nothing: times a hair past the last sample, and image values
+that are not finite where a trace's aperture or record leaves them out."""
 import numpy as np
 import pytest
 
@@ -26,3 +27,33 @@ def test_time_at_the_last_sample_reaches_no_other(nt, past):
     got, _ = gpu_demigrate(s, m)
     assert abs(got[0, -1] - 1.0) < 1e-3
     assert not np.any(got[0, :-1])
+
+
+def _masked(vel, aperture, nt=220):
+    rng = np.random.default_rng(9)
+    s = sv.survey_random(rng, 3, 200, 26, 19, 21, nt, vel=vel, weight="one", aperture=aperture, n_bins=2, h=12.5,
+                         v0=1700.0, k=0.5 if vel == "linear" else 0.0)
+    # shots of 40 receivers: warps of one, two and more source positions
+    pick = np.repeat(rng.permutation(s.ntr)[:5], 40)
+    s = s.replace(sx=s.sx[pick], sy=s.sy[pick])
+    off = np.hypot(s.sx.astype(np.float64) - s.rx, s.sy.astype(np.float64) - s.ry)
+    return s.replace(bin_width=(float(off.max()) * 1.0001 + 1.0) / s.n_bins)
+
+
+@pytest.mark.parametrize("vel", ["const", "linear"])
+@pytest.mark.parametrize("aperture, taper", [(0.0, 0.0), (90.0, 0.0), (90.0, 0.4)])
+@pytest.mark.parametrize("value", [np.nan, np.inf, -np.inf])
+def test_a_value_that_is_not_finite_stays_with_its_traces(vel, aperture, taper, value):
+    s = _masked(vel, aperture).replace(taper=taper)
+    m = sv.random_image(s, 3)
+    for p in ((0, 7, 11, 9), (1, 18, 25, 20), (0, 0, 0, 0)):
+        bad, base, unit = m.copy(), m.copy(), np.zeros_like(m)
+        bad[p], base[p], unit[p] = value, 0.0, 1.0
+        want, p1 = gpu_demigrate(s, base)
+        got, _ = gpu_demigrate(s, bad, plan=p1)
+        seen, _ = gpu_demigrate(s, unit, plan=p1)
+        hit = seen != 0.0   # samples the point adds to, and their neighbours (a weight of 0 there)
+        hit[:, 1:] |= seen[:, :-1] != 0.0
+        hit[:, :-1] |= seen[:, 1:] != 0.0
+        assert np.array_equal(got[~hit], want[~hit])
+        assert not np.all(np.isfinite(got[seen != 0.0])) or not np.any(seen)
