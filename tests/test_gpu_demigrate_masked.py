@@ -1,9 +1,11 @@
-"""The adjoint where a lane or a point is to add nothing: times a hair past the last sample, and image values
-that are not finite where a trace's aperture or record leaves them out."""
+"""The adjoint where a lane or a point is to add nothing: times a hair past the last sample, image values
+that are not finite where a trace leaves them out, and depths below the image where v0 + k z is no longer
+positive."""
 import numpy as np
 import pytest
 
-from helpers import gpu_demigrate
+import oracle
+from helpers import FP32_REL_L2, gpu_demigrate, rel_l2
 from paper_1204_1225_gb300 import survey as sv
 
 pytestmark = pytest.mark.gpu
@@ -57,3 +59,19 @@ def test_a_value_that_is_not_finite_stays_with_its_traces(vel, aperture, taper, 
         hit[:, :-1] |= seen[:, 1:] != 0.0
         assert np.array_equal(got[~hit], want[~hit])
         assert not np.all(np.isfinite(got[seen != 0.0])) or not np.any(seen)
+
+
+@pytest.mark.parametrize("weight", ["one", "obliq"])
+@pytest.mark.parametrize("v0", [300.0, 311.0])
+def test_depths_below_the_image_with_no_velocity(weight, v0):
+    # the image's last depth is the first of 32 in its tile, and v0 + k z reaches zero further down in it
+    dz, k, nz = 10.0, -0.5, 33
+    assert v0 + k * (nz - 1) * dz > 100.0 > 0.0 > v0 + k * 63 * dz
+    s = sv.survey_random(np.random.default_rng(7), 2, 70, 40, 1, nz, 300, vel="linear", weight=weight, n_bins=1, h=1.25,
+                         dt=0.05, v0=v0, k=k)
+    s = s.replace(dz=dz)
+    m = sv.random_image(s, 4)
+    got, _ = gpu_demigrate(s, m)
+    assert np.any(got)
+    # but for the two samples at each edge: a time within 2^-10 samples beyond it counts for the kernel alone
+    assert rel_l2(got[:, 2:-2], oracle.demigrate(s, m)[:, 2:-2]) < FP32_REL_L2
