@@ -676,6 +676,7 @@ __device__ __forceinline__ int mig_consumer(MigSmem& S, const TT* data, const Ge
         }
         const int cnt = S.cnt[s];
         const int last = S.last[s];
+        pf_t = -1;   // what was read ahead for a skipped trace of the last stage is no trace's of this one
         // a staged trace as this thread sees it
         struct View {
             int4 w;
