@@ -34,7 +34,8 @@ struct kh_batch_s {
     int n_items = 0;
     int ctas = 0;
     // The sorted work list is cut into parts of one ln(1 + rho) fit length each (shortest
-    // first); each part is one launch of the kernel compiled for that length.
+    // first); each part is one launch of the kernel compiled for that length (and for one part of the traces,
+    // where the partial images are not held).
     struct Part {
         int lg_terms, first, count, ctas;
     };
@@ -199,9 +200,10 @@ kh_status kirchhoff_batched_prepare(int njobs, const kh_job* jobs, kh_batch* out
     std::vector<CellGrid> cgs(njobs);
     size_t n_items = 0, n_cull = 0;
     size_t o_jobs = 0, o_items = 0, o_next = 0, o_status = 0, o_cull = 0;
-    // parts: traces cut into parts as the per-job calls cut them (left out where there is no room, as
-    // are the pairs of 16-bit traces)
-    auto lay_out = [&](bool parts, bool as_pairs) {
+    // Traces are cut into parts as the per-job calls cut them; held: with partial images of their own (where
+    // there is no room, a launch a part adds to the image, in the same order; the pairs of 16-bit traces are
+    // left out then)
+    auto lay_out = [&](bool held, bool as_pairs) {
         pairs = as_pairs;
         es = pairs ? (int)sizeof(SamplePair) : dtype_bytes((kh_dtype)tdt);
         ealign = 16 / es;
@@ -227,15 +229,15 @@ kh_status kirchhoff_batched_prepare(int njobs, const kh_job* jobs, kh_batch* out
             o.ld = o.padded ? (d.nt + ealign - 1) / ealign * ealign : d.nt;
             o.pad = o.padded ? L.take((size_t)J.ntr * o.ld * es) : 0;
             TileShape& t = tss[j];
-            // the per-job call's parts, with partial images of their own
-            t.split = parts && J.ntr > 0 ? split_of(gs[j], t, J.ntr) : 1;
-            o.split = t.split > 1 ? L.take((size_t)d.n_bins * d.ny * d.nx * d.nz * t.split * sizeof(float)) : 0;
+            t.split = J.ntr > 0 ? split_of(gs[j], t, J.ntr) : 1;
+            t.seq = t.split > 1 && !held ? 1 : 0;
+            o.split = t.split > 1 && held ? L.take((size_t)d.n_bins * d.ny * d.nx * d.nz * t.split * sizeof(float)) : 0;
             n_items += (size_t)t.tiles_x * t.tiles_y * t.tiles_z * d.n_bins * t.split;
             n_cull += (size_t)t.tiles_x * t.tiles_y * d.n_bins;
         }
         o_jobs = L.take(sizeof(BatchJob) * njobs);
         o_items = L.take(sizeof(int4) * n_items);
-        o_next = L.take(N_LG_TERMS * sizeof(int));
+        o_next = L.take(N_LG_TERMS * MAX_SPLIT * sizeof(int));
         o_status = L.take(sizeof(int));
         o_cull = L.take(sizeof(int) * std::max<size_t>(n_cull, 1));
     };
@@ -322,7 +324,7 @@ kh_status kirchhoff_batched_prepare(int njobs, const kh_job* jobs, kh_batch* out
             b->pads.push_back({J.ntr, d.nt, o.ld, es, J.traces, w + o.pad});
         }
         hj[j] = BatchJob{g, tss[j], tr, rows, J.image};
-        if (tss[j].split > 1) {
+        if (tss[j].split > 1 && !tss[j].seq) {
             hj[j].image = reinterpret_cast<float*>(w + o.split);
             b->sums.push_back({hj[j].image, tss[j].split, (long long)d.n_bins * d.ny * d.nx * d.nz, J.image});
             sum_of[j] = (int)b->sums.size() - 1;
@@ -341,8 +343,8 @@ kh_status kirchhoff_batched_prepare(int njobs, const kh_job* jobs, kh_batch* out
     if (e != cudaSuccess) return fail_free(set_cuda_error(e, "kirchhoff_batched_prepare: cull read-back"));
 
     // ---- work list: (job, tile, bin), estimated cost = points x (culled traces + 4).  Order:
-    // fit-length group (shortest first), then jobs by descending total cost, then bins, then
-    // longest item first.  Keeping a job's bin together keeps that bin's trace windows in L2
+    // part of the traces (where a launch takes one), fit-length group (shortest first), then jobs by
+    // descending total cost, then bins, then longest item first.  Keeping a job's bin together keeps that bin's trace windows in L2
     // while all CTAs work on it (as a per-job launch does); the smallest jobs form the tail.
     std::vector<int4> items(n_items);
     std::vector<double> cost(n_items);
@@ -365,7 +367,7 @@ kh_status kirchhoff_batched_prepare(int njobs, const kh_job* jobs, kh_batch* out
                         work += (double)cols * zs * c;
                         for (int part = 0; part < t.split; ++part, ++k) {
                             items[k] = make_int4(j, tile, bin, part);
-                            cls[k] = lg_class(gs[j].lg_terms);
+                            cls[k] = lg_class(gs[j].lg_terms) + (t.seq ? N_LG_TERMS * part : 0);
                             cost[k] = (double)cols * zs * ((double)c / t.split + 4);
                             job_cost[j] += cost[k];
                         }
@@ -432,11 +434,12 @@ kh_status kirchhoff_batched_prepare(int njobs, const kh_job* jobs, kh_batch* out
     gm.table = nullptr;
     b->g_max = gm;
     WaitCfg wc{b->d_status, b->wait_polls, WAIT_NS};
-    for (int c = 0, first = 0; c < N_LG_TERMS; ++c) {
-        int count = 0;
-        for (size_t i = 0; i < n_items; ++i) count += cls[i] == c ? 1 : 0;
+    int counts[N_LG_TERMS * MAX_SPLIT] = {};
+    for (size_t i = 0; i < n_items; ++i) ++counts[cls[i]];
+    for (int c = 0, first = 0; c < N_LG_TERMS * MAX_SPLIT; ++c) {   // by part, then by fit length
+        const int count = counts[c];
         if (count == 0) continue;
-        kh_batch_s::Part part{LG_TERMS[c], first, count, 0};
+        kh_batch_s::Part part{LG_TERMS[c % N_LG_TERMS], first, count, 0};
         e = launch_migrate_batched(gm, b->d_jobs, b->d_items + first, count, b->d_next + b->parts.size(), vel,
                                    weight, fast, part.lg_terms, kdt, wc, 0, &part.ctas, s);
         if (e != cudaSuccess) return fail_free(set_cuda_error(e, "kirchhoff_batched_prepare: kernel set-up"));
@@ -472,8 +475,11 @@ kh_status kirchhoff_migrate_batched(kh_batch b, void* cuda_stream)
                 if (e != cudaSuccess) return set_cuda_error(e, "kirchhoff_migrate_batched: row staging");
                 ++b->launches;
             }
-            e = launch_migrate(J.g, J.ts, J.tr, J.traces, J.image, b->vel, b->fast, wc, sk);
-            ++b->launches;
+            TileShape ts = J.ts;
+            do {   // one launch, or one a part
+                e = launch_migrate(J.g, ts, J.tr, J.traces, J.image, b->vel, b->fast, wc, sk);
+                ++b->launches;
+            } while (e == cudaSuccess && ts.seq && ++ts.seq <= ts.split);
             if (e == cudaSuccess && b->conc_sum[i] >= 0) {
                 const auto& m = b->sums[b->conc_sum[i]];
                 e = launch_split_sum(m.partial, m.split, m.n, m.image, sk);
@@ -495,7 +501,7 @@ kh_status kirchhoff_migrate_batched(kh_batch b, void* cuda_stream)
         ++b->launches;
     }
     if (b->n_items == 0) return KH_OK;
-    if ((e = cudaMemsetAsync(b->d_next, 0, N_LG_TERMS * sizeof(int), s)) != cudaSuccess)
+    if ((e = cudaMemsetAsync(b->d_next, 0, b->parts.size() * sizeof(int), s)) != cudaSuccess)
         return set_cuda_error(e, "kirchhoff_migrate_batched: counter reset");
     WaitCfg wc{b->d_status, b->wait_polls, WAIT_NS};
     for (size_t i = 0; i < b->parts.size(); ++i) {

@@ -192,10 +192,15 @@ struct TileShape {
     // Parts a tile's traces of a bin are cut into, each summed by a CTA of its own into a partial image
     // (the launch's image holds `split` of them; launch_split_sum adds them in order).
     int split = 1;
+    // 0: all parts in this launch; k + 1: part k alone, added to what the image holds (part 0 starts it).
+    // A batch's jobs: 1 where their work items add to the image, the parts in launches of their own.
+    int seq = 0;
 };
+constexpr int MAX_SPLIT = 32;
 
 // The number of parts for a launch of n_bins bins over ntr traces (by sizes alone, so that every path
-// that migrates the same job adds in the same order).
+// that migrates the same job adds in the same order; where the partial images cannot be held, the parts
+// are launched one after another).
 int split_of(const GeomParams& g, const TileShape& t, int ntr);
 
 struct WaitCfg {

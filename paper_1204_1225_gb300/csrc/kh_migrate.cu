@@ -99,7 +99,7 @@ int split_of(const GeomParams& g, const TileShape& t, int ntr)
     const double image = 4.0 * g.n_bins * g.ny * g.nx * (double)g.nz;
     int best = 1;
     double least = 1e300;
-    for (int s = 1; s <= 32 && (s == 1 || (per >= 16.0 * s && image * s <= 512e6)); ++s) {
+    for (int s = 1; s <= MAX_SPLIT && (s == 1 || (per >= 16.0 * s && image * s <= 512e6)); ++s) {
         const double waves = (double)((n * s + SLOTS - 1) / SLOTS);
         const double cost = waves * (per / s + 8.0) + (s > 1 ? 3.0 + s * image / 4e6 : 0.0);
         if (cost < (best == 1 ? 0.9 : 0.97) * least) {

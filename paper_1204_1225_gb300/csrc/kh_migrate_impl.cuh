@@ -595,7 +595,7 @@ template <int VEL, int WGT, bool FAST, typename TT, int LPT, typename TB>
 __device__ __forceinline__ int mig_consumer(MigSmem& S, const TT* data, const GeomParams& g,
                                             const TileShape& ts, int x0, int y0, int z0,
                                             const TileBox& box, int bin, float* __restrict__ image,
-                                            const WaitCfg& wc, const TB* tab, float2* srcc, int cap, int n)
+                                            const WaitCfg& wc, const TB* tab, float2* srcc, int cap, int n, bool add_to)
 {
     constexpr int WB = WGT & 3;                 // the weight (KH_W_*)
     constexpr bool AA = (WGT & W_AA) != 0;      // operator anti-aliasing compiled in
@@ -1081,6 +1081,12 @@ __device__ __forceinline__ int mig_consumer(MigSmem& S, const TT* data, const Ge
             a = make_float2(a.x * zg[i], a.y * zg[i + 1]);
             b = make_float2(b.x * zg[i + 2], b.y * zg[i + 3]);
         }
+        if (add_to) {   // the sum that k_split_sum forms, in the same order
+            if (izb + i < g.nz) a.x = __fadd_rn(out[i], a.x);
+            if (izb + i + 1 < g.nz) a.y = __fadd_rn(out[i + 1], a.y);
+            if (izb + i + 2 < g.nz) b.x = __fadd_rn(out[i + 2], b.x);
+            if (izb + i + 3 < g.nz) b.y = __fadd_rn(out[i + 3], b.y);
+        }
         if (vec) {
             *reinterpret_cast<float4*>(out + i) = make_float4(a.x, a.y, b.x, b.y);
         } else {
@@ -1392,10 +1398,11 @@ __device__ __forceinline__ void kernel_body(const GeomParams& g, const TileShape
     __syncthreads();
     if (s_abort) return;
     if (threadIdx.x >= CONSUMERS) {
-        mig_producer<VEL, TT, WGT>(S, data, cap, g, tr, traces, bin, box, wc, 0, (int)blockIdx.x, (int)blockIdx.z, ts.split);
+        mig_producer<VEL, TT, WGT>(S, data, cap, g, tr, traces, bin, box, wc, 0, (int)blockIdx.x,
+                                   ts.seq ? ts.seq - 1 : (int)blockIdx.z, ts.split);
     } else if constexpr (MODE == 0) {
         mig_consumer<VEL, WGT, FAST, TT, LPT, TB>(S, data, g, ts, x0, y0, z0, box, bin, image + split_offset(g, blockIdx.z),
-                                                  wc, tab, srcc, cap, 0);
+                                                  wc, tab, srcc, cap, 0, ts.seq > 1);
     } else {
         vg_consumer<VEL, WGT, FAST, TT, LPT>(S, data, g, ts, x0, y0, z0, box, bin, image, partial, wc, srcc, cap);
     }
@@ -1423,7 +1430,7 @@ static cudaError_t launch_migrate_t(const GeomParams& g, const TileShape& t, con
                                    const void* traces, float* image, const WaitCfg& w, cudaStream_t s)
 {
     const size_t smem = mig_smem_bytes(g);
-    const dim3 grid((unsigned)(t.tiles_x * t.tiles_y * t.tiles_z), (unsigned)g.n_bins, (unsigned)t.split);
+    const dim3 grid((unsigned)(t.tiles_x * t.tiles_y * t.tiles_z), (unsigned)g.n_bins, (unsigned)(t.seq ? 1 : t.split));
     auto go = [&](auto kern) -> cudaError_t {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -1615,8 +1622,8 @@ __global__ void __launch_bounds__(THREADS, 2)
                                       bin, box, wc, n, 0, w.w, ts.split);
         } else {
             n = mig_consumer<VEL, WGT, FAST, TT, LPT, float>(S, data, g, ts, x0, y0, z0, box, bin,
-                                                             jobs[w.x].image + split_offset(g, w.w), wc, nullptr, srcc,
-                                                             cap, n);
+                                                             jobs[w.x].image + (ts.seq ? 0 : split_offset(g, w.w)), wc,
+                                                             nullptr, srcc, cap, n, ts.seq && w.w > 0);
         }
     }
 }
