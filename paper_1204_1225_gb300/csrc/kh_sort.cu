@@ -263,6 +263,8 @@ __global__ void __launch_bounds__(SS_THREADS)
     }
 }
 
+bool sorts_in_one(int ntr) { return ntr <= SMALL_SORT; }
+
 cudaError_t sort_traces(int ntr, const float* sx, const float* sy, const float* rx, const float* ry,
                         int dim, int n_bins, double bin_width, const CellGrid& cg, int* key_a,
                         int* key_b, int* val_a, int* val_b, int* hist, int* cell_start, int* bin_start,
@@ -278,14 +280,14 @@ cudaError_t sort_traces(int ntr, const float* sx, const float* sy, const float* 
     if (ntr > 0) {
         k_cell_key<<<(ntr + 255) / 256, 256, 0, s>>>(ntr, sx, sy, rx, ry, dim, n_bins, bin_width, cg, kin, vin);
         ++*launches;
-        if (ntr <= SMALL_SORT) {
+        if (sorts_in_one(ntr)) {
             const cudaError_t e = cudaFuncSetAttribute(k_small_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                        (int)sizeof(SmallSortSmem));
             if (e != cudaSuccess) return e;
             k_small_sort<<<1, SS_THREADS, sizeof(SmallSortSmem), s>>>(ntr, kin, passes, nkeys, ncell, sx, sy, rx, ry,
-                                                                       dim, vout, cell_start, bin_start, hdr, mid);
+                                                                       dim, vin, cell_start, bin_start, hdr, mid);
             ++*launches;
-            *perm_out = vout;
+            *perm_out = vin;
             return cudaGetLastError();
         }
         for (int p = 0; p < passes; ++p) {
