@@ -6,7 +6,9 @@ of the weighted offset images across the bins, V(v0, k).  Its gradient comes fro
 kernels alone: the semblance kernel writes dV/dI, and the velocity-gradient kernel turns it into
 dV/d(v0, k) = d<dV/dI, L(v0, k) D>/d(v0, k).  ``VelocityAnalysis.run`` minimises V with a BFGS
 iteration on scaled parameters and an Armijo backtracking line search (host logic on two
-numbers; every image and gradient is computed on the device).
+numbers; every image and gradient is computed on the device).  A trial model that the library does not
+take (KH_ERR_INVALID_ARG or KH_ERR_UNSUPPORTED: v(z) not positive over the image, windows too long)
+halves the step like one that does not decrease V.
 """
 from __future__ import annotations
 
@@ -44,7 +46,9 @@ class VelocityAnalysis:
 
     def run(self, v0: float, k: float, n_iter: int = 30, scale=(100.0, 0.1), tol: float = 1e-12):
         """Minimises V from (v0, k): BFGS on (v0 / scale[0], k / scale[1]).  Returns a dict with
-        the final model, V and the history of (v0, k, V)."""
+        the final model, V and the history of (v0, k, V).  Ends at the last accepted model where the
+        library refuses every step down to 1e-3 of a search direction; a refused start, or a first search
+        refused throughout, raises the library's error, as any other error does at once."""
         sc = np.asarray(scale, dtype=np.float64)
         th = np.array([v0, k], dtype=np.float64)
         V, g0, g1 = self.objective(*th)
@@ -53,20 +57,28 @@ class VelocityAnalysis:
         hist = [(float(th[0]), float(th[1]), V)]
         for _ in range(n_iter):
             p = -Hinv @ g
-            a = 1.0
+            a, refused = 1.0, False
             while True:   # Armijo backtracking
                 tn = th + a * p * sc
                 try:
                     Vn, h0, h1 = self.objective(*tn)
                 except kh.KirchhoffError as e:
-                    # the quasi-Newton step left the models the library takes: a shorter step
-                    if e.status not in (kh.KH_ERR_UNSUPPORTED, kh.KH_ERR_INVALID_ARG) or a < 1e-3:
+                    # the quasi-Newton step left the models the library takes (which took the start, with
+                    # the same headers and traces): a shorter step
+                    if e.status not in (kh.KH_ERR_UNSUPPORTED, kh.KH_ERR_INVALID_ARG):
                         raise
+                    if a < 1e-3:
+                        if len(hist) == 1:
+                            raise
+                        refused = True
+                        break
                     a *= 0.5
                     continue
                 if Vn <= V + 1e-4 * a * float(g @ p) or a < 1e-3:
                     break
                 a *= 0.5
+            if refused:
+                break
             gn = np.array([h0, h1]) * sc
             step, y = a * p, gn - g
             sy = float(step @ y)
