@@ -467,9 +467,7 @@ __device__ __forceinline__ int mig_producer(MigSmem& S, TT* data, int cap, const
                     const double rsc = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(esx, esx), __dmul_rn(esy, esy)), zc2));
                     const double rrc = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(erx, erx), __dmul_rn(ery, ery)), zc2));
                     tau_ref = __dadd_rn(tau_ref, __ddiv_rn(__dadd_rn(rsc, rrc), __dmul_rn(g.v0, g.dtd)));
-                    // and what the reference loses when it is rounded to FP32, as a length
-                    const double rel = tau_ref - (double)lo;
-                    S.refs[s][slot] = make_float4((float)rsc, (float)rrc, (float)((rel - (double)(float)rel) * (g.v0 * g.dtd)), 0.f);
+                    S.refs[s][slot] = make_float4((float)rsc, (float)rrc, 0.f, 0.f);
                     S.hda[s][slot] = make_float4((float)(box.cx - 2.0 * h.x), (float)(box.cy - 2.0 * h.y),
                                                  (float)(box.cx - 2.0 * h.z), (float)(box.cy - 2.0 * h.w));
                     }
@@ -591,11 +589,26 @@ __device__ __forceinline__ void thread_column(const TileShape& ts, int tid, int&
 // changes.  tau - lo = c0rel + C1 ln(1 + rho_s) + C1 ln(1 + rho_r) with c0rel = tau_ref - lo,
 // each leg's logarithm from the per-leg fit (LPT = its length).  The weight's gamma(z)
 // multiplies each depth's sum once, before the store.
+// Adds a column's depths to the parts before: the sum that k_split_sum forms, in the same order.  A call for
+// linear v(z), where these lines in the kernel cost every launch 0.5 % (10 000 traces into 256^3: 140.5 -> 141.1
+// ms), and in the kernel else, where the call costs (radial tables 1.5 %).
+__device__ __forceinline__ void add_column_here(float* out, int n, float4 a, float4 b, float4 c, float4 d)
+{
+    const float v[16] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w, d.x, d.y, d.z, d.w};
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+        if (i < n) out[i] = __fadd_rn(out[i], v[i]);
+}
+__device__ __noinline__ static void add_column(float* out, int n, float4 a, float4 b, float4 c, float4 d)
+{
+    add_column_here(out, n, a, b, c, d);
+}
+
 template <int VEL, int WGT, bool FAST, typename TT, int LPT, typename TB>
 __device__ __forceinline__ int mig_consumer(MigSmem& S, const TT* data, const GeomParams& g,
                                             const TileShape& ts, int x0, int y0, int z0,
                                             const TileBox& box, int bin, float* __restrict__ image,
-                                            const WaitCfg& wc, const TB* tab, float2* srcc, int cap, int n, bool add_to)
+                                            const WaitCfg& wc, const TB* tab, float2* srcc, int cap, int n)
 {
     constexpr int WB = WGT & 3;                 // the weight (KH_W_*)
     constexpr bool AA = (WGT & W_AA) != 0;      // operator anti-aliasing compiled in
@@ -926,9 +939,7 @@ __device__ __forceinline__ int mig_consumer(MigSmem& S, const TT* data, const Ge
                 // two-way time, hundreds of samples, is in the FP64 reference).  One reciprocal root
                 // gives 1/R_a and R_a = q_a / R_a; the source leg's (dR_s, 1/R_s) is cached per source
                 // position.  The weight z (R_s + R_r) (1/R_s^2 + 1/R_r^2) / 2 (2D: sqrt(R_s R_r)) is 0 on
-                // the surface row, where zc's z / 2 is stored as 0 (every factor is finite, see root_pair).  What the
-                // FP32 reference c0rel leaves out joins the receiver leg's FMA: without it the image of 10 000 traces
-                // (151 x 133 x 117 points, aperture 800 m) is off by 1.16e-6, with it by 0.91e-6 (15.55 -> 15.71 ms)
+                // the surface row, where zc's z / 2 is stored as 0 (every factor is finite, see root_pair)
                 int aacls = 1;   // anti-aliasing classes as in the direct branch
                 if constexpr (AA) {
                     aacls = aa_class(g.aa_c, cxf - h.x, cyf - h.y, cxf - h.z, cyf - h.w, aa_lo, aa_hi, inside);
@@ -950,13 +961,13 @@ __device__ __forceinline__ int mig_consumer(MigSmem& S, const TT* data, const Ge
                     psy = __float_as_uint(h.y);
                 }
                 struct Leg {
-                    F2 dP, dh2, rc, lo, c0;
+                    F2 dP, dh2, rc, c0;
                 };
                 auto leg = [&](int tt, const View& q) -> Leg {
-                    const float4 a = S.hda[s][tt], rf = S.refs[s][tt];   // rf: (R_sc, R_rc, the reference's low part, -)
+                    const float4 a = S.hda[s][tt];
                     const float ex = cxf - q.h.z, ey = cyf - q.h.w;
-                    return Leg{f2(fmaf(dxc, cxf + a.z, dyc * (cyf + a.w))), f2(fmaf(ex, ex, ey * ey)), f2(rf.y), f2(rf.z),
-                               f2(__int_as_float(q.w.x))};
+                    return Leg{f2(fmaf(dxc, cxf + a.z, dyc * (cyf + a.w))), f2(fmaf(ex, ex, ey * ey)), f2(S.refs[s][tt].y),
+                               f2(__int_as_float(q.w.x))};   // refs: (R_sc, R_rc, -, -)
                 };
                 F2 ir_last = 0;   // 1/R_r of the depth pair evaluated last
                 auto eval = [&](const Leg& q) {
@@ -966,7 +977,7 @@ __device__ __forceinline__ int mig_consumer(MigSmem& S, const TT* data, const Ge
                         F2 Rr, ir;
                         root_pair<FAST>(add2(q.dh2, c.x), Rr, ir);
                         if constexpr (AA) ir_last = ir;
-                        const F2 dR = fma2(add2(q.dP, c.y), rcp2<FAST>(max2(add2(Rr, q.rc), 1e-30f)), q.lo);
+                        const F2 dR = mul2(add2(q.dP, c.y), rcp2<FAST>(max2(add2(Rr, q.rc), 1e-30f)));
                         const F2 is = sv.y, qs = add2(dhs2, c.x), Rs = FAST ? mul2(qs, is) : sqrt2<false>(qs);
                         const F2 amp = g.dim == 3 ? add2(Rs, Rr) : sqrt2<FAST>(mul2(Rs, Rr));
                         W = mul2(mul2(zc[2 * p + 1].x, amp), fma2(is, is, mul2(ir, ir)));
@@ -1074,18 +1085,25 @@ __device__ __forceinline__ int mig_consumer(MigSmem& S, const TT* data, const Ge
     float* out = image + (((long long)bin * g.ny + iy) * g.nx + ix) * (long long)g.nz + izb;
     const bool vec = ((g.nz & 3) == 0) && (izb + NZ <= g.nz) &&
                      ((reinterpret_cast<uintptr_t>(image) & 15) == 0);
+    if (ts.seq > 1) {   // a part of its own launch
+        float4 q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float2 a = f2_get(acc[2 * i]), b = f2_get(acc[2 * i + 1]);
+            q[i] = make_float4(a.x, a.y, b.x, b.y);
+            if constexpr (WB == 1)
+                q[i] = make_float4(a.x * zg[4 * i], a.y * zg[4 * i + 1], b.x * zg[4 * i + 2], b.y * zg[4 * i + 3]);
+        }
+        if constexpr (VEL == VK_LINEAR) add_column(out, g.nz - izb, q[0], q[1], q[2], q[3]);
+        else add_column_here(out, g.nz - izb, q[0], q[1], q[2], q[3]);
+        return n;
+    }
 #pragma unroll
     for (int i = 0; i < NZ; i += 4) {
         float2 a = f2_get(acc[i / 2]), b = f2_get(acc[i / 2 + 1]);
         if constexpr (WB == 1) {
             a = make_float2(a.x * zg[i], a.y * zg[i + 1]);
             b = make_float2(b.x * zg[i + 2], b.y * zg[i + 3]);
-        }
-        if (add_to) {   // the sum that k_split_sum forms, in the same order
-            if (izb + i < g.nz) a.x = __fadd_rn(out[i], a.x);
-            if (izb + i + 1 < g.nz) a.y = __fadd_rn(out[i + 1], a.y);
-            if (izb + i + 2 < g.nz) b.x = __fadd_rn(out[i + 2], b.x);
-            if (izb + i + 3 < g.nz) b.y = __fadd_rn(out[i + 3], b.y);
         }
         if (vec) {
             *reinterpret_cast<float4*>(out + i) = make_float4(a.x, a.y, b.x, b.y);
@@ -1402,7 +1420,7 @@ __device__ __forceinline__ void kernel_body(const GeomParams& g, const TileShape
                                    ts.seq ? ts.seq - 1 : (int)blockIdx.z, ts.split);
     } else if constexpr (MODE == 0) {
         mig_consumer<VEL, WGT, FAST, TT, LPT, TB>(S, data, g, ts, x0, y0, z0, box, bin, image + split_offset(g, blockIdx.z),
-                                                  wc, tab, srcc, cap, 0, ts.seq > 1);
+                                                  wc, tab, srcc, cap, 0);
     } else {
         vg_consumer<VEL, WGT, FAST, TT, LPT>(S, data, g, ts, x0, y0, z0, box, bin, image, partial, wc, srcc, cap);
     }
@@ -1605,7 +1623,8 @@ __global__ void __launch_bounds__(THREADS, 2)
         if (it >= n_items) break;
         const int4 w = items[it];
         const GeomParams g = jobs[w.x].g;
-        const TileShape ts = jobs[w.x].ts;
+        TileShape ts = jobs[w.x].ts;
+        if (ts.seq) ts.seq = w.w + 1;
         const TraceSet tr = jobs[w.x].tr;
         int t = w.y;
         const int tzi = t % ts.tiles_z;
@@ -1623,7 +1642,7 @@ __global__ void __launch_bounds__(THREADS, 2)
         } else {
             n = mig_consumer<VEL, WGT, FAST, TT, LPT, float>(S, data, g, ts, x0, y0, z0, box, bin,
                                                              jobs[w.x].image + (ts.seq ? 0 : split_offset(g, w.w)), wc,
-                                                             nullptr, srcc, cap, n, ts.seq && w.w > 0);
+                                                             nullptr, srcc, cap, n);
         }
     }
 }
